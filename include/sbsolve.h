@@ -263,27 +263,36 @@ typedef struct {
 } sb_shape;
 
 /* The shape solves with this factor's (half bandwidth, N), arithmetic and dtypes
- * will use: a stored entry if there is one, else the built-in default for a large batch.
- * Without an entry an FP64 solve in native arithmetic takes the two-ended sweeps, or the
- * FP64 partitioned solve where the batch is small, if the matrix may be eliminated in any
- * order (diagonally dominant by rows or columns, or symmetric positive definite), and
- * the sequential sweeps otherwise.  Without an entry an FP32 right-hand side of up to 128
- * rows takes the sequential sweeps with every system held in registers (the same bits),
- * which no shape names; batches of at most two 32-system tiles an SM stay partitioned
- * from 65 rows on. */
+ * will use: a stored entry if there is one, else the one that stands for the built-in
+ * default, which is a rule on the batch:
+ *   FP64 in native arithmetic: the two-ended sweeps, or the FP64 partitioned solve where
+ *     the batch is small, if the matrix may be eliminated in any order (diagonally
+ *     dominant by rows or columns, or symmetric positive definite), and the sequential
+ *     sweeps otherwise;
+ *   FP32 right-hand sides: up to 128 rows the sequential sweeps with every system held in
+ *     registers (the same bits), except that batches of at most two 32-system tiles an SM
+ *     stay partitioned from 65 rows on; beyond 128 rows the partitioned solve.
+ * The shape that stands for the default is that of a large batch, with ctas_per_sm = 1
+ * where one CTA fills an SM anyway. */
 int sb_shape_get(const sb_factor* f, sb_arith arith, sb_dtype rhs_dtype, sb_dtype x_dtype,
                  sb_shape* out);
 
 /* Store a shape for that key (process-wide, on the factor's device); for example
- * one loaded from a tuning cache.  SB_ERR_INVALID_ARG for an out-of-range shape. */
+ * one loaded from a tuning cache.  It holds for batches of every size.  Storing the shape
+ * that stands for the default (sb_shape_get without an entry, or sb_autotune where the
+ * default was fastest) drops the entry, so that the rule above applies again; ask for that
+ * kernel alone, whatever the batch, with ctas_per_sm = 0.  SB_ERR_INVALID_ARG for an
+ * out-of-range shape. */
 int sb_shape_set(const sb_factor* f, sb_arith arith, sb_dtype rhs_dtype, sb_dtype x_dtype,
                  const sb_shape* shape);
 
 /*
- * sb_autotune -- time every candidate shape (sequential: threads 64..512, CTAs/SM
- * 0..2, systems per thread 1..2; partitioned, where it applies) on the caller's buffers with CUDA events (one warm-up
- * and the best of three launches each), store the fastest as for sb_shape_set and
- * return it in *best (and its time in *best_ms; either may be NULL).  x is
+ * sb_autotune -- time the built-in default and every candidate shape (sequential: threads
+ * 64..512, CTAs/SM 0..2, systems per thread 1..2; staged, two-ended and partitioned, where
+ * they apply) on the caller's buffers with CUDA events (one warm-up and the best of three
+ * launches each), store the fastest as for sb_shape_set and return it in *best (and its
+ * time in *best_ms; either may be NULL).  Where no shape beats the default by 2 % the
+ * entry is dropped and *best is the shape that stands for the default.  x is
  * overwritten and must differ from rhs; arguments otherwise as for
  * sb_solve_batched_ex.  Blocking: it synchronises on `stream`.  The autotuner is
  * this library's own (the paper's kernels have a fixed one-thread-per-system shape).

@@ -246,6 +246,7 @@ int resident_run(const sb_stepper* st, double* state, int64_t M, int64_t ld, int
                  cudaStream_t stream);
 // FP32 solves of systems of up to kRegMaxRows rows held in registers (sweep_reg.cu).
 constexpr int kRegMaxRows = 128;
+constexpr int kRegThreads = 128;
 bool reg_sweep_applies(const sb_factor* f, sb_dtype rt, sb_dtype xt, sb_arith arith);
 int launch_reg_sweep(const sb_factor* f, Op op, const void* rhs, void* x, sb_dtype xt, int64_t M, int64_t ld,
                      cudaStream_t stream);

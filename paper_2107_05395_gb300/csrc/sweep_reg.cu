@@ -22,8 +22,6 @@
 namespace sb {
 namespace {
 
-constexpr int kRegThreads = 128;
-
 template <typename T, int n>
 struct alignas(sizeof(T) * n) RegVec {
   T v[n];

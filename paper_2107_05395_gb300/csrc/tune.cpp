@@ -5,8 +5,15 @@
 // from sb_shape_set (e.g. a persisted tuning cache) or from sb_autotune, which
 // times every candidate shape on the caller's buffers with CUDA events and keeps
 // the fastest.  Without an entry, FP32 right-hand sides in native arithmetic use the
-// register-resident sweeps up to 128 rows and the partitioned solve where it applies, FP64 ones the two-ended sweeps or, for a small
-// batch, the FP64 partitioned solve, and everything else the default of sweep.cu.
+// register-resident sweeps up to 128 rows and the partitioned solve where it applies,
+// FP64 ones the two-ended sweeps or, for a small batch, the FP64 partitioned solve, and
+// everything else the default of sweep.cu.
+//
+// That default is a rule on M and alignment, and some of its forms no shape names, so it
+// cannot be an entry: the shape that stands for it (default_route of a large batch) is
+// never stored, and storing it drops the entry instead.  Where an explicit request for the
+// same kernel is possible, the two differ in ctas_per_sm: 1 in the default, 0 in a
+// request, which run alike because one such CTA fills an SM.
 #include <algorithm>
 #include <map>
 #include <mutex>
@@ -53,34 +60,31 @@ bool fp64_shape(const sb_factor* f, Op op, int64_t M, SweepShape* s) {
   for (int threads : {1024, 512, 256})
     if (two_ended_applies(f, op, SB_ARITH_NATIVE, threads)) {
       s->threads = threads;
+      s->ctas_per_sm = 1;  // all that fit
       s->algo = SB_ALGO_TWO_ENDED;
       return true;
     }
   return false;
 }
 
-}  // namespace
-
-SweepShape shape_for(const sb_factor* f, Op op, sb_arith arith, sb_dtype rt, sb_dtype xt, int64_t M) {
-  std::lock_guard<std::mutex> lk(g_mu);
-  auto it = g_table.find(make_key(f, arith, rt, xt));
-  if (it != g_table.end()) return it->second;
+// The shape a solve of M systems takes without a stored entry.
+SweepShape default_route(const sb_factor* f, Op op, sb_arith arith, sb_dtype rt, sb_dtype xt, int64_t M) {
+  SweepShape s;
+  const bool reg = reg_sweep_applies(f, rt, xt, arith);
   // FP32 right-hand sides in native arithmetic default to the partitioned solve where
   // the factor has its data (the launcher falls back to the sweeps per call where it
   // does not apply)
   if (arith == SB_ARITH_NATIVE && rt == SB_F32 && (f->part_img[0][0] || f->part_img[1][0])) {
-    SweepShape s;
     // two systems per thread (variant 2) where the factor has its image
     s.threads = (f->part_img[0][2] || f->part_img[1][2]) ? 256 : 512;
-    s.ctas_per_sm = 0;
-    s.spt = 1;
+    s.ctas_per_sm = 1;  // all that fit
     s.algo = SB_ALGO_PARTITIONED;
-    s.reg = reg_sweep_applies(f, rt, xt, arith);
+    s.reg = reg;
     return s;
   }
-  SweepShape s;
-  if (reg_sweep_applies(f, rt, xt, arith)) {
+  if (reg) {
     s = default_shape(f, arith);
+    s.threads = kRegThreads;
     s.reg = true;
     return s;
   }
@@ -98,6 +102,28 @@ SweepShape shape_for(const sb_factor* f, Op op, sb_arith arith, sb_dtype rt, sb_
   return default_shape(f, arith);
 }
 
+bool same_shape(const SweepShape& a, const SweepShape& b) {
+  return a.threads == b.threads && a.ctas_per_sm == b.ctas_per_sm && a.spt == b.spt && a.algo == b.algo;
+}
+
+void copy_shape(const SweepShape& s, sb_shape* out) {
+  out->threads = s.threads;
+  out->ctas_per_sm = s.ctas_per_sm;
+  out->systems_per_thread = s.spt;
+  out->algorithm = s.algo;
+}
+
+}  // namespace
+
+SweepShape shape_for(const sb_factor* f, Op op, sb_arith arith, sb_dtype rt, sb_dtype xt, int64_t M) {
+  {
+    std::lock_guard<std::mutex> lk(g_mu);
+    auto it = g_table.find(make_key(f, arith, rt, xt));
+    if (it != g_table.end()) return it->second;
+  }
+  return default_route(f, op, arith, rt, xt, M);
+}
+
 }  // namespace sb
 
 using namespace sb;
@@ -108,11 +134,7 @@ int sb_shape_get(const sb_factor* f, sb_arith arith, sb_dtype rhs_dtype, sb_dtyp
                  sb_shape* out) {
   clear_error();
   if (!f || !out) return fail(SB_ERR_INVALID_ARG, "NULL argument");
-  const SweepShape s = shape_for(f, OP_PRIMAL, arith, rhs_dtype, x_dtype, kLargeBatch);
-  out->threads = s.threads;
-  out->ctas_per_sm = s.ctas_per_sm;
-  out->systems_per_thread = s.spt;
-  out->algorithm = s.algo;
+  copy_shape(shape_for(f, OP_PRIMAL, arith, rhs_dtype, x_dtype, kLargeBatch), out);
   return SB_OK;
 }
 
@@ -148,8 +170,12 @@ int sb_shape_set(const sb_factor* f, sb_arith arith, sb_dtype rhs_dtype, sb_dtyp
   s.ctas_per_sm = shape->ctas_per_sm;
   s.spt = shape->systems_per_thread;
   s.algo = shape->algorithm;
+  const bool is_default = same_shape(s, default_route(f, OP_PRIMAL, arith, rhs_dtype, x_dtype, kLargeBatch));
   std::lock_guard<std::mutex> lk(g_mu);
-  g_table[make_key(f, arith, rhs_dtype, x_dtype)] = s;
+  if (is_default)
+    g_table.erase(make_key(f, arith, rhs_dtype, x_dtype));
+  else
+    g_table[make_key(f, arith, rhs_dtype, x_dtype)] = s;
   return SB_OK;
 }
 
@@ -173,9 +199,13 @@ int sb_autotune(const sb_factor* f, int transpose, const void* rhs, sb_dtype rhs
     cudaEventDestroy(e0);
     return rc;
   }
-  SweepShape winner = default_shape(f, arith);
+  // The default route first.  It adapts to every batch and a stored entry does not, so a
+  // shape has to beat it by 2 % (above the spread of three launches) to be stored.
+  const SweepShape route = default_route(f, op, arith, rhs_dtype, x_dtype, M);
+  SweepShape winner = route;
   float winner_ms = 1e30f;
-  std::vector<SweepShape> cands;
+  bool route_wins = true;
+  std::vector<SweepShape> cands{route};
   for (int spt : {1, 2})
     for (int threads : {64, 128, 256, 512})
       for (int cps : {0, 1, 2}) {
@@ -237,24 +267,25 @@ int sb_autotune(const sb_factor* f, int transpose, const void* rhs, sb_dtype rhs
       clear_error();
       continue;
     }
-    if (ms_best < winner_ms) {
+    const bool is_route = &s == cands.data();
+    if (is_route || ms_best < (route_wins ? 0.98f : 1.0f) * winner_ms) {
       winner_ms = ms_best;
       winner = s;
+      route_wins = is_route;
     }
   }
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);
   if (winner_ms >= 1e30f) return fail(SB_ERR_CUDA, "no candidate shape could be launched");
+  if (route_wins) winner = default_route(f, OP_PRIMAL, arith, rhs_dtype, x_dtype, kLargeBatch);
   {
     std::lock_guard<std::mutex> lk(g_mu);
-    g_table[make_key(f, arith, rhs_dtype, x_dtype)] = winner;
+    if (route_wins)
+      g_table.erase(make_key(f, arith, rhs_dtype, x_dtype));
+    else
+      g_table[make_key(f, arith, rhs_dtype, x_dtype)] = winner;
   }
-  if (best) {
-    best->threads = winner.threads;
-    best->ctas_per_sm = winner.ctas_per_sm;
-    best->systems_per_thread = winner.spt;
-    best->algorithm = winner.algo;
-  }
+  if (best) copy_shape(winner, best);
   if (best_ms) *best_ms = winner_ms;
   return SB_OK;
 }
