@@ -349,22 +349,8 @@ int launch_fused(const sb_stepper* st, const typename A::C* coef, const typename
                 "N=%d too large for the fused step's shared memory (only FP64 steps read the "
                 "coefficients from device memory)", N);
   const int threads = 256;
-  static std::mutex mu;
-  static std::map<std::pair<const void*, int>, int> occ;
   int nb = 0;
-  {
-    std::lock_guard<std::mutex> lk(mu);
-    auto key = std::make_pair(reinterpret_cast<const void*>(k), (int)smem);
-    auto it = occ.find(key);
-    if (it == occ.end()) {
-      SB_CUDA(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxDynSmem));
-      SB_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k, threads, smem));
-      occ[key] = nb;
-    } else {
-      nb = it->second;
-    }
-  }
-  if (nb < 1) return fail(SB_ERR_UNSUPPORTED, "fused step kernel cannot be resident");
+  SB_TRY(kernel_occupancy(reinterpret_cast<const void*>(k), f->device, threads, smem, &nb));
   const int64_t ntiles = (M + 31) / 32;
   const int64_t grid = std::max<int64_t>(1, std::min<int64_t>(ntiles, (int64_t)nb * sm_count(f->device)));
   const typename A::C* cy = CYC ? StepCyc<A>::rows(f) : nullptr;  // primal rows (op 0)

@@ -13,9 +13,10 @@
 // writes the solution over it.  Rows are fetched R at a time into registers with
 // double buffering: the next batch is in flight while the current one is swept.
 #include <algorithm>
-#include <type_traits>
+#include <map>
 #include <mutex>
-#include <unordered_map>
+#include <tuple>
+#include <type_traits>
 
 #include "sb_internal.h"
 #include "sweep_tile.cuh"
@@ -607,12 +608,13 @@ int dispatch_pb(const sb_factor* f, Op op, const typename A::C* base, const void
 
 namespace {
 std::mutex g_occ_mu;
-std::unordered_map<uint64_t, int> g_occ;
+std::map<std::tuple<const void*, int, int, size_t>, int> g_occ;
 }  // namespace
 
+// The shared-memory attribute below belongs to (kernel, device), so the device is part of
+// the key: a kernel's first launch on another device has to set it there too.
 int kernel_occupancy(const void* kernel, int device, int threads, size_t smem, int* blocks_per_sm) {
-  const uint64_t key = (reinterpret_cast<uint64_t>(kernel) * 31u) ^ ((uint64_t)smem << 20) ^
-                       ((uint64_t)threads << 8) ^ (uint64_t)device;
+  const auto key = std::make_tuple(kernel, device, threads, smem);
   {
     std::lock_guard<std::mutex> lk(g_occ_mu);
     auto it = g_occ.find(key);
