@@ -202,10 +202,10 @@ int sb_solve_batched_ex(const sb_factor* f, int transpose, const void* rhs, sb_d
  *                        element written once.  It applies to FP32 rhs with FP32 or FP64
  *                        x in native arithmetic, 64 <= N <= 1024, rhs 16-byte aligned
  *                        and ld a multiple of 4, when every chunk's factorisation has
- *                        non-zero pivots.  Rows aligned otherwise are copied without
- *                        TMA where that is faster than the sequential sweeps and the
- *                        matrix may be eliminated in any order; elsewhere a solve asked
- *                        to use it runs the sequential sweeps with their default shape.
+ *                        non-zero pivots; elsewhere a solve asked to use it runs the
+ *                        sequential sweeps with their default shape, or (rows aligned
+ *                        otherwise, where it is faster) the same sweeps of systems held
+ *                        in shared memory, with the same bits.
  *                        With 128-thread CTAs it is the FP64 form for latency-bound
  *                        batches: tiles of 8 systems cut into 16 chunks of 8/16/32 rows
  *                        (32 <= N <= 512), FP64 rhs and x, native arithmetic, the

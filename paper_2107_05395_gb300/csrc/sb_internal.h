@@ -250,6 +250,11 @@ constexpr int kRegThreads = 128;
 bool reg_sweep_applies(const sb_factor* f, sb_dtype rt, sb_dtype xt, sb_arith arith);
 int launch_reg_sweep(const sb_factor* f, Op op, const void* rhs, void* x, sb_dtype xt, int64_t M, int64_t ld,
                      cudaStream_t stream);
+// FP32 solves of systems held in shared memory, with the bits of the sequential sweeps
+// (sweep_chip.cu): for right-hand sides that the partitioned solve cannot copy.
+bool chip_sweep_applies(const sb_factor* f, sb_dtype rt, sb_dtype xt, int64_t M, sb_arith arith);
+int launch_chip_sweep(const sb_factor* f, Op op, const void* rhs, void* x, sb_dtype xt, int64_t M, int64_t ld,
+                      cudaStream_t stream);
 // The partitioned solve (partition.cu); shape.algo == SB_ALGO_PARTITIONED.
 // The small-tile FP64 partitioned solve (partition64.cu): 128-thread CTAs, 16 chunks.
 constexpr int kPart64Threads = 128;
@@ -265,11 +270,6 @@ bool partitioned_applies(const sb_factor* f, Op op, const void* rhs, sb_dtype rh
                          sb_dtype x_dtype, int64_t M, int64_t ld, sb_arith arith, int threads);
 // Reads and resets the count of partitioned-solve CTAs that timed out on `device`.
 int partition_timeouts(int device, unsigned* count);
-// The same for right-hand sides that TMA cannot copy (rows not 16-byte aligned).
-bool partitioned_rows_applies(const sb_factor* f, Op op, sb_dtype rhs_dtype, sb_dtype x_dtype, int64_t M,
-                              sb_arith arith);
-int launch_partitioned_rows(const sb_factor* f, Op op, const void* rhs, void* x, sb_dtype x_dtype, int64_t M,
-                            int64_t ld, cudaStream_t stream);
 int launch_partitioned(const sb_factor* f, Op op, const void* rhs, sb_dtype rhs_dtype, void* x,
                        sb_dtype x_dtype, int64_t M, int64_t ld, sb_arith arith,
                        const SweepShape& shape, cudaStream_t stream);

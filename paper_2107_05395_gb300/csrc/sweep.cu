@@ -670,10 +670,11 @@ int launch_sweep(const sb_factor* f, Op op, const void* rhs, sb_dtype rhs_dtype,
   if (shape.algo == SB_ALGO_PARTITIONED) {
     if (partitioned_applies(f, op, rhs, rhs_dtype, x_dtype, M, ld, arith, shape.threads))
       return launch_partitioned(f, op, rhs, rhs_dtype, x, x_dtype, M, ld, arith, shape, stream);
-    if (partitioned_rows_applies(f, op, rhs_dtype, x_dtype, M, arith))
-      return launch_partitioned_rows(f, op, rhs, x, x_dtype, M, ld, stream);
-    // where the partition does not apply (sizes, dtypes) the sequential sweeps run with
-    // their default shape
+    // where the partition does not apply (sizes, dtypes, alignment) the sequential sweeps
+    // run, of systems held on chip where that is faster (the same bits), else with their
+    // default shape
+    if (chip_sweep_applies(f, rhs_dtype, x_dtype, M, arith))
+      return launch_chip_sweep(f, op, rhs, x, x_dtype, M, ld, stream);
     return launch_sweep(f, op, rhs, rhs_dtype, x, x_dtype, M, ld, arith, default_shape(f, arith),
                         stream);
   }
