@@ -342,7 +342,8 @@ int sb_build_matrix(int kind, int64_t N, double coef, double* diags);
  * each chunk is copied to the device, solved and copied back on one of three
  * internal streams, so both copy directions overlap the solves of neighbouring
  * chunks.  Asynchronous: the work is ordered after prior work on `stream` and
- * `stream` waits for all of it (synchronise it before reading x_host).
+ * `stream` waits for all of it (synchronise it before reading x_host).  Without a stored
+ * shape the chunk size does not change the bits of the solution.
  *   rhs_host, x_host  host arrays in the N x ld interleaved layout (may be the same
  *                     array); page-locked memory is needed for the copies to overlap.
  *   work              caller-owned device workspace of sb_host_workspace_bytes() bytes.

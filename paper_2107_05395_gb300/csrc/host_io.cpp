@@ -108,8 +108,7 @@ int sb_solve_batched_host(const sb_factor* f, int transpose, const void* rhs_hos
   const int64_t N = f->N;
   const size_t slot = host_slot_bytes(N, C, rs, xs), x_off = host_slot_x_offset(N, C, rs);
   const Op op = transpose ? OP_ADJOINT : OP_PRIMAL;
-  // the large batch's shape whatever M is, so that the chunk size does not change the bits
-  const SweepShape shape = shape_for(f, op, arith, rhs_dtype, x_dtype, kLargeBatch);
+  const SweepShape shape = shape_for_pieces(f, op, arith, rhs_dtype, x_dtype);
   int64_t chunk = 0;
   for (int64_t m0 = 0; m0 < M; m0 += C, ++chunk) {
     const int64_t Mc = std::min(C, M - m0);

@@ -62,7 +62,9 @@ struct SweepShape {
   int ctas_per_sm = 0;   // cap on resident CTAs per SM (0 = occupancy limit)
   int spt = 1;           // systems per thread (1 or 2)
   int algo = SB_ALGO_SEQUENTIAL;  // sequential sweeps or the partitioned solve
-  bool reg = false;      // systems whole in registers instead (sweep_reg.cu; never a stored shape)
+  // FP32 systems held whole in registers (sweep_reg.cu) or in shared memory (sweep_chip.cu)
+  // instead; never part of a stored shape
+  bool reg = false, chip = false;
 };
 
 // Partitioned-solve variants: variant v cuts the rows into part_chunks(v) chunks:
@@ -228,6 +230,9 @@ bool two_ended_applies(const sb_factor* f, Op op, sb_arith arith, int threads);
 // for a batch of M systems.
 constexpr int64_t kLargeBatch = INT64_MAX;
 SweepShape shape_for(const sb_factor* f, Op op, sb_arith arith, sb_dtype rt, sb_dtype xt, int64_t M);
+// The same for a batch that is solved in pieces: without a stored entry a shape whose form
+// depends on neither a piece's M nor its alignment, so that the cut does not show in the bits.
+SweepShape shape_for_pieces(const sb_factor* f, Op op, sb_arith arith, sb_dtype rt, sb_dtype xt);
 // One fused stepper step from src into dst (stepper.cu).
 int stepper_step(const sb_stepper* st, const double* src, double* dst, int64_t M, int64_t ld,
                  sb_arith arith, cudaStream_t stream);
@@ -252,6 +257,9 @@ int launch_reg_sweep(const sb_factor* f, Op op, const void* rhs, void* x, sb_dty
                      cudaStream_t stream);
 // FP32 solves of systems held in shared memory, with the bits of the sequential sweeps
 // (sweep_chip.cu): for right-hand sides that the partitioned solve cannot copy.
+// fits: the systems have a place there; applies: and a batch of M is faster so than in the
+// sequential sweeps.
+bool chip_sweep_fits(const sb_factor* f, sb_dtype rt, sb_dtype xt, sb_arith arith);
 bool chip_sweep_applies(const sb_factor* f, sb_dtype rt, sb_dtype xt, int64_t M, sb_arith arith);
 int launch_chip_sweep(const sb_factor* f, Op op, const void* rhs, void* x, sb_dtype xt, int64_t M, int64_t ld,
                       cudaStream_t stream);

@@ -661,6 +661,8 @@ int launch_sweep(const sb_factor* f, Op op, const void* rhs, sb_dtype rhs_dtype,
       !(f->N > 64 && M <= 2 * 32 * (int64_t)sm_count(f->device) && shape.algo == SB_ALGO_PARTITIONED &&
         partitioned_applies(f, op, rhs, rhs_dtype, x_dtype, M, ld, arith, shape.threads)))
     return launch_reg_sweep(f, op, rhs, x, x_dtype, M, ld, stream);
+  if (shape.chip && chip_sweep_fits(f, rhs_dtype, x_dtype, arith))
+    return launch_chip_sweep(f, op, rhs, x, x_dtype, M, ld, stream);
   if (shape.algo == SB_ALGO_PARTITIONED && shape.threads == kPart64Threads) {
     if (partitioned64_applies(f, op, rhs_dtype, x_dtype, M, arith))
       return launch_partitioned64(f, op, rhs, x, M, ld, shape, stream);

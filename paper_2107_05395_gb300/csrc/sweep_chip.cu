@@ -198,6 +198,11 @@ int launch(const sb_factor* f, const float* coef, const float* rhs, TO* x, int64
 
 }  // namespace
 
+bool chip_sweep_fits(const sb_factor* f, sb_dtype rt, sb_dtype xt, sb_arith arith) {
+  return arith == SB_ARITH_NATIVE && rt == SB_F32 && (xt == SB_F32 || xt == SB_F64) && !f->periodic &&
+         chip_bytes(f) <= (size_t)kMaxDynSmem;
+}
+
 // Against the sequential sweeps: always faster with an FP64 solution, whose FP32
 // intermediate takes 8-byte places there.  With an FP32 solution those sweeps catch up once
 // they have enough warps to hide their latency and the intermediate still finds place in
@@ -206,11 +211,9 @@ int launch(const sb_factor* f, const float* coef, const float* rhs, TO* x, int64
 // 30 | 29, M = 120001 41 | 50; N = 1000 M = 20001 167 | 86, M = 60001 217 | 213,
 // pentadiagonal 225 | 242).
 bool chip_sweep_applies(const sb_factor* f, sb_dtype rt, sb_dtype xt, int64_t M, sb_arith arith) {
-  if (arith != SB_ARITH_NATIVE || rt != SB_F32 || f->periodic || M < 1) return false;
-  const size_t bytes = chip_bytes(f);
-  if (bytes > (size_t)kMaxDynSmem) return false;
-  const int64_t warps = 2 * bytes <= (size_t)kMaxDynSmem ? 16 : 10;
-  return xt == SB_F64 || (xt == SB_F32 && M <= 32 * warps * sm_count(f->device));
+  const int64_t warps = 2 * chip_bytes(f) <= (size_t)kMaxDynSmem ? 16 : 10;
+  return chip_sweep_fits(f, rt, xt, arith) && M >= 1 &&
+         (xt == SB_F64 || M <= 32 * warps * sm_count(f->device));
 }
 
 int launch_chip_sweep(const sb_factor* f, Op op, const void* rhs, void* x, sb_dtype xt, int64_t M, int64_t ld,

@@ -124,6 +124,20 @@ SweepShape shape_for(const sb_factor* f, Op op, sb_arith arith, sb_dtype rt, sb_
   return default_route(f, op, arith, rt, xt, M);
 }
 
+SweepShape shape_for_pieces(const sb_factor* f, Op op, sb_arith arith, sb_dtype rt, sb_dtype xt) {
+  SweepShape s = shape_for(f, op, arith, rt, xt, kLargeBatch);
+  // FP32: registers or partition by a piece's M, TMA or not by its width.  The sequential
+  // sweeps on chip are one form for all (the copies to and from the host take several times
+  // as long as any of them).
+  if (rt == SB_F32 && same_shape(s, default_route(f, op, arith, rt, xt, kLargeBatch))) {
+    const bool reg = s.reg;
+    s = default_shape(f, arith);
+    s.reg = reg;
+    s.chip = !reg;
+  }
+  return s;
+}
+
 }  // namespace sb
 
 using namespace sb;
