@@ -25,6 +25,7 @@
 // chunk side by side), so a coefficient read is one conflict-free 256-byte access.
 #include <algorithm>
 #include <cmath>
+#include <mutex>
 #include <type_traits>
 #include <vector>
 
@@ -305,10 +306,50 @@ int dispatch(const sb_stepper* st, double* state, int64_t M, int64_t ld, int64_t
 
 }  // namespace
 
-int build_resident(sb_stepper* st, const std::vector<double>& erows) {
+namespace {
+
+// The batch up to which these steps beat the one-thread-per-simulation ones, with chunks of
+// L rows and NL reduction levels.  Those take a latency of about N (430 + 71 n) cycles for n
+// FP64 operations a row, whatever the batch; these take 17 cycles of an SM's FP64 unit per
+// operation of each simulation's warp.  Microseconds per step there | here (the rule's line
+// for M):
+//   diffusion, CN, periodic, N = 256:  M = 4096 124 | 21, 16384 132 | 79, 32768 146 | 156 (21700)
+//   hyperdiffusion, CN, periodic, N = 100:  M = 4096 70 | 55, 8192 70 | 105 (4600)
+//   Cahn-Hilliard, no flux, N = 512:  M = 8192 261 | 134, 16384 275 | 269 (10700)
+int64_t batch_limit(const sb_stepper* st, int L, int NL) {
+  const int PB = st->fac->P, Q = 2 * PB, rank = st->fac->periodic ? st->fac->periodic_rank : 0;
+  const int row_there = 2 * PB + 2 * rank + (st->has_e ? 5 : st->NB);
+  const int row_here = 1 + 2 * PB + Q + rank + (st->has_e ? 5 : st->NB > 0 ? 1 : 0);
+  const int ops = L * row_here + Q * Q + NL * (Q * Q + 2 * Q * PB) + 6 * rank;
+  return (int64_t)(0.9 * sm_count(st->fac->device) * st->N * (430.0 + 71.0 * row_there) / (17.0 * ops));
+}
+
+// A device copy of `img`, made on a stream of its own in relaxed capture mode: the first
+// small batch may be stepped inside a capture of the caller's, or while another thread
+// captures.
+int upload(const std::vector<double>& img, double** out) {
+  cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+  SB_CUDA(cudaThreadExchangeStreamCaptureMode(&mode));
+  double* d = nullptr;
+  cudaStream_t s = nullptr;
+  const size_t bytes = img.size() * sizeof(double);
+  cudaError_t e = cudaMalloc(&d, bytes);
+  if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking);
+  if (e == cudaSuccess) e = cudaMemcpyAsync(d, img.data(), bytes, cudaMemcpyHostToDevice, s);
+  if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+  if (s != nullptr) cudaStreamDestroy(s);
+  if (e != cudaSuccess && d != nullptr) cudaFree(d);
+  cudaThreadExchangeStreamCaptureMode(&mode);
+  SB_TRY(cuda_check(e, "image of the on-chip steps"));
+  *out = d;
+  return SB_OK;
+}
+
+// The image, made by the first small batch that is stepped (most steppers never see one).
+int build_resident(sb_stepper* st) {
+  const std::vector<double>& erows = st->e_rows;
   const sb_factor* f = st->fac;
   const int PB = f->P, N = (int)f->N, L = chunk_rows(f->N), Q = 2 * PB;
-  if (f->N < kLanes || L == 0 || !f->any_order) return SB_OK;
   Partition p;
   if (!build_partition(PB, N, f->h_diag.data(), L, kLanes, p)) return SB_OK;
   const int K = p.K();
@@ -352,28 +393,27 @@ int build_resident(sb_stepper* st, const std::vector<double>& erows) {
       }
     }
   }
-  DeviceGuard g(f->device);
-  SB_TRY(g.rc);
-  SB_CUDA(cudaMalloc(&st->res_img, img.size() * sizeof(double)));
+  SB_TRY(upload(img, &st->res_img));
   st->res_L = L;
   st->res_NL = NL;
-  // The batch up to which these steps beat the one-thread-per-simulation ones.  Those
-  // take a latency of about N (430 + 71 n) cycles for n FP64 operations a row, whatever
-  // the batch; these take 17 cycles of an SM's FP64 unit per operation of each
-  // simulation's warp.  Microseconds per step there | here (the rule's line for M):
-  //   diffusion, CN, periodic, N = 256:  M = 4096 124 | 21, 16384 132 | 79, 32768 146 | 156 (21700)
-  //   hyperdiffusion, CN, periodic, N = 100:  M = 4096 70 | 55, 8192 70 | 105 (4600)
-  //   Cahn-Hilliard, no flux, N = 512:  M = 8192 261 | 134, 16384 275 | 269 (10700)
-  const int row_there = 2 * PB + 2 * rank + (st->has_e ? 5 : st->NB);
-  const int row_here = 1 + 2 * PB + Q + rank + (st->has_e ? 5 : st->NB > 0 ? 1 : 0);
-  const int ops = L * row_here + Q * Q + NL * (Q * Q + 2 * Q * PB) + 6 * rank;
-  st->res_max_M = (int64_t)(0.9 * sm_count(f->device) * N * (430.0 + 71.0 * row_there) / (17.0 * ops));
-  return cuda_check(cudaMemcpy(st->res_img, img.data(), img.size() * sizeof(double), cudaMemcpyHostToDevice),
-                    "cudaMemcpy");
+  st->res_max_M = batch_limit(st, L, NL);
+  return SB_OK;
 }
 
-bool resident_applies(const sb_stepper* st, int64_t M, sb_arith arith) {
-  return st->res_img != nullptr && arith == SB_ARITH_NATIVE && M <= st->res_max_M;
+}  // namespace
+
+int resident_applies(sb_stepper* st, int64_t M, sb_arith arith, bool* applies) {
+  *applies = false;
+  const sb_factor* f = st->fac;
+  const int L = chunk_rows(f->N);
+  if (arith != SB_ARITH_NATIVE || f->N < kLanes || L == 0 || !f->any_order || M > batch_limit(st, L, 0)) return SB_OK;
+  std::lock_guard<std::mutex> lk(st->mu);
+  if (!st->res_built) {
+    SB_TRY(build_resident(st));
+    st->res_built = true;
+  }
+  *applies = st->res_img != nullptr && M <= st->res_max_M;
+  return SB_OK;
 }
 
 int resident_run(const sb_stepper* st, double* state, int64_t M, int64_t ld, int64_t nsteps, cudaStream_t s) {

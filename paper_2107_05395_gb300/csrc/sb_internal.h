@@ -177,8 +177,11 @@ struct sb_stepper {
   double* s64 = nullptr;
   int s64_fast = 0, s64_ka = 0, s64_kb = 0;
   bool s64_third = false;
-  // resident.cu: image of the on-chip steps of small batches (null where they do not
-  // apply), its chunk length and reduction levels, and the largest batch that takes them
+  // resident.cu: image of the on-chip steps of small batches (made by the first such batch;
+  // null where they do not apply), its chunk length and reduction levels, and the largest
+  // batch that takes them
+  std::vector<double> e_rows;  // host: the E rows of a Cahn-Hilliard stepper
+  bool res_built = false;
   double* res_img = nullptr;
   int res_L = 0, res_NL = 0;
   int64_t res_max_M = 0;
@@ -243,10 +246,9 @@ int step64(const sb_stepper* st, const double* src, double* state, int64_t M, in
            cudaStream_t stream, double* ellm = nullptr);
 int step64_forced(const sb_stepper* st, double* state, const double* amp, int64_t M, int64_t ld,
                   cudaStream_t stream);
-// Steps of a small batch kept on chip (resident.cu): the image (built with the stepper;
-// erows: the E rows of a Cahn-Hilliard stepper), whether a batch takes them, and the run.
-int build_resident(sb_stepper* st, const std::vector<double>& erows);
-bool resident_applies(const sb_stepper* st, int64_t M, sb_arith arith);
+// Steps of a small batch kept on chip (resident.cu): whether a batch takes them (the first
+// that may makes their image, also inside a capture), and the run.
+int resident_applies(sb_stepper* st, int64_t M, sb_arith arith, bool* applies);
 int resident_run(const sb_stepper* st, double* state, int64_t M, int64_t ld, int64_t nsteps,
                  cudaStream_t stream);
 // FP32 solves of systems of up to kRegMaxRows rows held in registers (sweep_reg.cu).

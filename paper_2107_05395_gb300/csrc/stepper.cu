@@ -612,7 +612,7 @@ int sb_stepper_create(int kind, int scheme, int bc, int64_t N, double coef, doub
     }
   }
   rc = build_step64(st, rows);
-  if (rc == SB_OK) rc = build_resident(st, rows);
+  if (st->has_e) st->e_rows = std::move(rows);
   if (rc != SB_OK) {
     sb_stepper_destroy(st);
     return rc;
@@ -823,7 +823,9 @@ int sb_stepper_run(sb_stepper* st, double* state, int64_t M, int64_t ld, sb_arit
     return SB_OK;
   }
 
-  if (resident_applies(st, M, arith)) return resident_run(st, state, M, ld, nsteps, s);
+  bool on_chip = false;
+  SB_TRY(resident_applies(st, M, arith, &on_chip));
+  if (on_chip) return resident_run(st, state, M, ld, nsteps, s);
 
   // graphs of kGraphSteps fused steps, replayed; the remainder launched directly
   const auto key = std::make_tuple(reinterpret_cast<uintptr_t>(state), M, ld, (int)arith, kGraphSteps);
