@@ -2,10 +2,15 @@
 // down (host C++ only).  The two-ended and partitioned solves take no pivots in orders
 // that the plain factorisation of A says nothing about: a matrix whose LU is harmless
 // can have a tiny pivot from the other end or inside a chunk.  For the two classes
-// below every order is stable without pivoting (growth at most 2, and pivots no
-// smaller than A's own), so those solves may be taken without being asked for:
-//   * weakly diagonally dominant by rows or by columns, with a non-zero diagonal;
-//   * symmetric positive definite (symmetric, and every pivot of A = LU positive).
+// below every order is stable without pivoting, so those solves may be taken without
+// being asked for:
+//   * weakly diagonally dominant by rows or by columns, with a non-zero diagonal: what is
+//     left after any row is eliminated is dominant again, and no entry grows beyond twice
+//     the largest of A;
+//   * symmetric positive definite (symmetric, and every pivot of A = LU positive): nothing
+//     grows, and no pivot is smaller than A's smallest eigenvalue.
+// The pivots themselves differ from one order to another: [[1, 1], [1, 2]] has 1, 1 from
+// the first row down and 2, 1/2 from the last row up.
 #pragma once
 
 #include <cmath>
