@@ -272,6 +272,10 @@ typedef struct {
  *   FP32 right-hand sides: up to 128 rows the sequential sweeps with every system held in
  *     registers (the same bits), except that batches of at most two 32-system tiles an SM
  *     stay partitioned from 65 rows on; beyond 128 rows the partitioned solve.
+ * These rules look at M and at the alignment of the call, and their forms eliminate in
+ * different orders: the bits of a system's solution depend on the batch it is solved in (a
+ * shard or a slice of a batch agrees with the whole to rounding).  SB_ALGO_SEQUENTIAL,
+ * SB_ALGO_STAGED or (FP64) SB_ALGO_TWO_ENDED, stored, is one form for every batch.
  * The shape that stands for the default is that of a large batch, with ctas_per_sm = 1
  * where one CTA fills an SM anyway. */
 int sb_shape_get(const sb_factor* f, sb_arith arith, sb_dtype rhs_dtype, sb_dtype x_dtype,
