@@ -36,8 +36,11 @@ N_ROWS = 1024
 M_SYS = 65536
 R_COEF = 0.25
 SEED = 2
-# FP64 flops per element of one pentadiagonal solve: forward 2 FMA + 1 MUL, backward 2 FMA.
-FLOPS_PER_ELT = 9
+# flops of the FP64 pipe per element of one pentadiagonal solve: forward 2 FMA, backward 2
+# FMA (the forward scaling, a ninth flop of the algorithm, runs on the integer pipes)
+FLOPS_PER_ELT = 8
+# flops of the algorithm per element (what double-float arithmetic does in other operations)
+SOLVE_FLOPS_PER_ELT = 9
 BYTES_PER_ELT = 16  # read the RHS once, write the solution once (FP64)
 SM_COUNT = 152
 SM_MAX_GHZ = 2.07
@@ -684,8 +687,10 @@ def summary(extras, fp32, df32, cpu, timeouts, link=None, fp64_fma_per_s=None):
     the end of the JSON line): times in ms (table1 in s per 1000 steps), fractions
     of the measured HBM peak, ratios against the plain per-step solve, the host
     link's copy rates (GB/s) beside the end-to-end figure, and the refined
-    multi-group solve against its FP64-pipe bound (8 FP64 operations per element:
-    3 FMAs per residual row and 1 addition per correction, two passes)."""
+    multi-group solve against the FP64-pipe bound of two residuals and corrections in
+    FP64 (8 operations per element: 3 FMAs per residual row and 1 addition per
+    correction, two passes; the kernel does 5, the first residual in FP32 pairs and a
+    correction on the integer pipes, so the ratio can pass 1)."""
     ch = extras.get("cahn_hilliard", {})
     mg = extras.get("multigroup_refine", {})
     ro = extras.get("adjoint_rollout", {})
@@ -924,6 +929,7 @@ def run_ours(args):
     elts = N_ROWS * M_SYS
     flops = FLOPS_PER_ELT * elts
     achieved_tflops = flops / avg_launch_s / 1e12
+    equiv_tflops = SOLVE_FLOPS_PER_ELT * elts / avg_launch_s / 1e12
     hbm, hbm_src = hbm_peak()
     achieved_gbs = BYTES_PER_ELT * elts / avg_launch_s / 1e9
     traffic = profiled_traffic()
@@ -955,7 +961,7 @@ def run_ours(args):
                 "frac": achieved_gbs / hbm, "traffic": traffic,
                 "kernel": headline_kernel("DFArith", "double-float arithmetic, FP64 I/O"),
                 "peak_source": f"{hbm_src} (MEASURED_PEAKS.json hbm_gbs)",
-                "alu_fp64_equiv": {"achieved": achieved_tflops, "unit": "TFLOP/s"}}
+                "alu_fp64_equiv": {"achieved": equiv_tflops, "unit": "TFLOP/s"}}
         dtype = "f64 (double-float arithmetic)"
     else:
         roof = {"bound": "alu", "achieved": achieved_tflops, "peak": fp64_peak,

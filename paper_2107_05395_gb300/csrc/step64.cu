@@ -18,12 +18,15 @@
 //     unit is not);
 //   * the WENO term shares differences between rows and divides once, by Newton's
 //     iteration from a single-precision reciprocal (see Weno).
-// FP64 operations a row, before and now, and a step (FP64 unit busy, now):
-//   Crank-Nicolson diffusion, periodic, N = 1024, M = 65536:  7, 4.2 (6 near the ends);
-//     0.996 -> 0.624 ms (87 %)
-//   Cahn-Hilliard without flux, N = 256, M = 2^20:  9, 8;  4.06 -> 3.58 ms
-//   periodic, with the coarsening length, N = 256, M = 65536:  14, 11;  0.428 -> 0.343 ms
-//   forced, N = 512, M = 98304:  86, 40;  9.18 -> 4.18 ms (84 %)
+// FP64 operations a row (counted on the device), before and now, and a step (of the cycles
+// of an SM that has work, those its FP64 unit is busy, now):
+//   Crank-Nicolson diffusion, periodic, N = 1024, M = 65536:  7, 4.8 (4 without periodic
+//     ends; the correction's rows are 0.2 of the rest, and the dot product of every other
+//     batch of the others is issued under a false predicate, 0.5);  0.996 -> 0.624 ms (87 %)
+//   Cahn-Hilliard without flux, N = 256, M = 2^20:  9, 8;  4.06 -> 3.58 ms (94 %)
+//   periodic, with the coarsening length, N = 256, M = 65536:  14, 11.1;  0.428 -> 0.343 ms (94 %)
+//   forced, N = 512, M = 98304:  86, 40.4;  9.18 -> 4.18 ms (80 %; 8 to 40 bytes of its
+//     registers spill, 0.03 loads a row)
 #include <algorithm>
 #include <cmath>
 #include <cstring>
@@ -143,6 +146,8 @@ struct Weno {
     const double t2 = fma(e2, e2, fma(13.0 / 3.0, s[1], eps));
     const double t3 = fma(e3, e3, fma(13.0 / 3.0, s[2], eps));
     // t are positive (>= 4e-99): their high words order like their exponents
+    // (infinite only where a difference exceeds 1e153: phi of such a C has overflowed too and
+    // takes the whole simulation with it, whatever W comes to)
     const int top = max(max(__double2hiint(t1), __double2hiint(t2)), __double2hiint(t3));
     const int k = 1023 - (top >> 20);
     const double r1 = scale2(t1, k), r2 = scale2(t2, k), r3 = scale2(t3, k);

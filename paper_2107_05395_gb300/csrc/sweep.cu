@@ -106,7 +106,8 @@ sweep_staged_kernel(const typename A::C* __restrict__ coef, int N, int64_t M, in
 // (mulc_fast): the four products of a batch have one test between them, so they overlap
 // each other and the FP64 unit; with a test and a branch in each product a warp took
 // 500 cycles a row for one FP64 operation of 64.  Bound: the FP64 unit for pentadiagonal
-// systems (N = 1024, M = 65536: 480 -> 452 us of a 428 us bound), DRAM for tridiagonal
+// systems (N = 1024, M = 65536: 480 -> 457 us of a 428 us bound, the unit busy 95 % of the
+// time; 4 and 12 bytes of the 64 registers spill, 0.002 loads a row), DRAM for tridiagonal
 // ones whose intermediate leaves L2 (the same size: 399 -> 318 us, 2.1 GB), the latency of
 // the rows for small batches (tridiagonal, N = 511, M = 30011: 125 -> 92 us; M = 1024:
 // 77 -> 44 us).
@@ -177,12 +178,13 @@ struct Ends64 {
 
 // Double-float: the image after the FP64 one holds the same values as (hi, lo) pairs.
 // Both conversions test a batch at once, like the products above: a conversion with its
-// own branch is a scheduling barrier between rows, and the sweep is bound by issue (67 %
+// own branch is a scheduling barrier between rows, and the sweep is bound by issue (66 %
 // of the slots at N = 512, M = 65536, pentadiagonal: 174 us, 259 with one-ended sweeps;
-// 128 instructions an element, where DRAM would take 79 us for its 16 bytes).
+// 127 instructions an element, where DRAM would take 79 us for its 16 bytes).  At 72
+// registers 28 bytes (tridiagonal) and 40 spill, 0.05 loads an element; 64 spill more.
 template <int P>
 struct EndsDf {
-  static constexpr int kMaxThreads = 448, kMinCtas = 2;  // 72 registers; 64 spill
+  static constexpr int kMaxThreads = 448, kMinCtas = 2;  // 72 registers
   using V = df;
   using Pre = df;  // F0
   using Row = TwoRowDf<P>;
