@@ -354,8 +354,6 @@ SB_HD df double_to_df(double v) {
     const uint32_t fb = bb | ((lo >> 6) & 0x7FFFFFu);
     return {u2f(hb), f_sub(u2f(fb), u2f(bb))};
   }
-  // zeros (point sources, padded states) without the FP64 unit and the call: the same pair
-  if (((hi & 0x7FFFFFFFu) | lo) == 0u) return {u2f(hi), 0.f};
   return double_to_df_slow(v);  // exact fallback (rare)
 }
 

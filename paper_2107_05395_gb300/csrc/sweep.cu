@@ -181,7 +181,29 @@ struct Ends64 {
 // own branch is a scheduling barrier between rows, and the sweep is bound by issue (66 %
 // of the slots at N = 512, M = 65536, pentadiagonal: 174 us, 259 with one-ended sweeps;
 // 127 instructions an element, where DRAM would take 79 us for its 16 bytes).  At 72
-// registers 28 bytes (tridiagonal) and 40 spill, 0.05 loads an element; 64 spill more.
+// registers 20 bytes (tridiagonal) and 40 spill, 0.05 loads an element; 64 spill more.
+struct DfBatch {
+  df v[kTwoBatch];
+};
+// A batch with a value that the branchless split does not take, out of line as a whole: one
+// call for the batch, and its zeros (point sources, padded states) need no FP64 unit.  N =
+// 512, M = 65536, tridiagonal, point sources: 405 -> 225 us with four calls -> this (dense
+// 168); a test for zeros in every conversion cost dense double-float steps 2 %.
+__device__ __noinline__ DfBatch double_to_df_batch(double b0, double b1, double b2, double b3) {
+  static_assert(kTwoBatch == 4);
+  const double b[kTwoBatch] = {b0, b1, b2, b3};
+  DfBatch r;
+#pragma unroll
+  for (int j = 0; j < kTwoBatch; ++j) {
+    r.v[j] = double_to_df_fast(b[j]);
+    if (((d_hi(b[j]) & 0x7FFFFFFFu) | d_lo(b[j])) == 0u)
+      r.v[j] = df{u2f(d_hi(b[j])), 0.f};
+    else if (!double_to_df_ok(b[j]))
+      r.v[j] = double_to_df_slow(b[j]);  // a call, or its FP64 operations would run for all
+  }
+  return r;
+}
+
 template <int P>
 struct EndsDf {
   static constexpr int kMaxThreads = 448, kMinCtas = 2;  // 72 registers
@@ -203,8 +225,10 @@ struct EndsDf {
       s[j] = double_to_df_fast(b[j]);
     }
     if (!ok) {
+      static_assert(K == kTwoBatch);
+      const DfBatch r = double_to_df_batch(b[0], b[1], b[2], b[3]);
 #pragma unroll
-      for (int j = 0; j < K; ++j) s[j] = double_to_df(b[j]);
+      for (int j = 0; j < K; ++j) s[j] = r.v[j];
     }
   }
   static __device__ __forceinline__ V forward(const Pre* p, const Row& c, V s, V v1, V v2) {
