@@ -8,18 +8,19 @@
 // against FP64 in the median of 195 matrices, 1.32 times at most.)
 //
 // One warp of a CTA sweeps; its time is the chain of 2 N rows, so it does nothing else: the
-// other three copy the tile in and the solution out, a quarter of the rows behind or ahead
-// of it, and refill the rows of a stored quarter with the next tile's.  Every element is
-// copied, stored and replaced by the same thread, and the four quarters change hands at
-// barriers of the CTA.  A system's rows lie in fours, so that the sweeping warp reads and
-// writes 16 bytes at a time: with 4-byte accesses it took 25 ns a row, now 12 (17 a
-// pentadiagonal one).
+// others copy the tile in and the solution out, a quarter of the rows behind or ahead
+// of it.  The backward sweep is done with the last quarter first, and the next tile needs
+// its first quarter first: it goes into the place of the last, so quarters lie in turn
+// upwards and downwards.  A quarter changes hands at a barrier of the CTA, and a place is
+// stored and refilled by the same warp.  A system's rows lie in fours, so that the sweeping
+// warp reads and writes 16 bytes at a time: with 4-byte accesses it took 25 ns a row, now
+// 10 (12 a pentadiagonal one).
 //
 // Microseconds, sequential | partitioned with cp.async | this form (chip_sweep_applies
-// draws the line): tridiagonal N = 1000: M = 501 134 | 13.3 | 19.9, M = 60001 217 | 138 |
-// 213; N = 256: M = 6001 37.5 | 11.6 | 13.2, M = 60001 52 | 51 | 41; pentadiagonal N = 512:
-// M = 6001 77 | 19 | 21, M = 20001 88 | 36 | 43; with an FP64 solution, tridiagonal N = 130,
-// M = 240001 184 | 123 | 98, pentadiagonal N = 256, M = 60001 76 | 66 | 49.
+// draws the line): tridiagonal N = 1000: M = 501 134 | 13.3 | 21, M = 20001 167 | 55 | 80;
+// N = 256: M = 6001 38 | 11.6 | 12.4, M = 60001 52 | 51 | 41; pentadiagonal N = 512: M = 6001
+// 77 | 19 | 20, M = 20001 88 | 36 | 41; with an FP64 solution, tridiagonal N = 130, M =
+// 240001 184 | 123 | 90, pentadiagonal N = 256, M = 60001 76 | 66 | 51.
 #include <algorithm>
 #include <cstdint>
 #include <type_traits>
@@ -30,7 +31,6 @@
 namespace sb {
 namespace {
 
-constexpr int kChipThreads = 128;
 constexpr int kChipBatch = 8;  // rows the sweeping warp reads at once
 constexpr int kChipParts = 4;
 
@@ -41,14 +41,19 @@ struct alignas(P == 1 ? 8 : 16) ChipRec {
   float v[W];
 };
 
+// Rows of a quarter.
+__host__ __device__ inline int chip_part(int N) {
+  return ((N + kChipParts - 1) / kChipParts + kChipBatch - 1) / kChipBatch * kChipBatch;
+}
+
 __device__ __forceinline__ void cp_row4(float* dst, const float* src) {
   asm volatile("cp.async.ca.shared.global.L2::256B [%0], [%1], 4;\n" ::"r"(shared_addr(dst)),
                "l"(__cvta_generic_to_global(src))
                : "memory");
 }
 
-template <int P, bool F_ONE, bool B_ONE, typename TO>
-__global__ void __launch_bounds__(kChipThreads)
+template <int P, bool F_ONE, bool B_ONE, typename TO, int T>
+__global__ void __launch_bounds__(T)
 sweep_chip_kernel(const float* __restrict__ coef, int N, int64_t M, int64_t ld, const float* rhs, TO* x,
                   int64_t ntiles, int sms) {
   using F = NativeArith<float>;
@@ -60,27 +65,31 @@ sweep_chip_kernel(const float* __restrict__ coef, int N, int64_t M, int64_t ld, 
   Rec* cs = reinterpret_cast<Rec*>(smem_raw);  // forward rows, then (NP rows on) backward rows
   const int lane = threadIdx.x & 31;
   float4* const col = reinterpret_cast<float4*>(cs + 2 * NP) + lane;  // four rows of this lane's system each
-  auto at = [&](int i) -> float* { return reinterpret_cast<float*>(col + (i >> 2) * 32) + (i & 3); };
   // CTAs of one SM have block indices about `sms` apart: their sweeping warps go to
-  // different schedulers.  role 0 sweeps, 1 to 3 copy.
-  const int role = ((threadIdx.x >> 5) + (int)(blockIdx.x / sms)) & 3;
-  const int part = ((N + kChipParts - 1) / kChipParts + R - 1) / R * R;  // rows of a quarter, whole batches
-  const int last = (N + part - 1) / part - 1;                            // quarters that have rows: 0 .. last
+  // different schedulers.  role 0 sweeps, 1 to nw - 1 copy.
+  constexpr int nw = T / 32;  // 4 or 8
+  const int role = ((threadIdx.x >> 5) + (int)(blockIdx.x / sms)) & (nw - 1);
+  const int part = chip_part(N);               // rows of a quarter, whole batches
+  const int last = (N + part - 1) / part - 1;  // quarters that have rows: 0 .. last
   auto end = [&](int q) { return min(N, (q + 1) * part); };
-  auto fill = [&](int64_t m, int first, int q, int step) {  // this warp's rows of a quarter
+  // how far a quarter's rows lie from their own places: none, or (down) in reverse order
+  auto shift = [&](int q, bool down) { return down ? (last - 2 * q) * part : 0; };
+  auto at = [&](int i) -> float* { return reinterpret_cast<float*>(col + (i >> 2) * 32) + (i & 3); };
+  auto fill = [&](int64_t m, int first, int q, int step, bool down) {  // this warp's rows of a quarter
     if (m < M) {
+      const int off = shift(q, down);
       const float* src = rhs + m + (int64_t)(q * part + first) * ld;
 #pragma unroll 4
-      for (int i = q * part + first; i < end(q); i += step, src += step * ld) cp_row4(at(i), src);
+      for (int i = q * part + first; i < end(q); i += step, src += step * ld) cp_row4(at(i + off), src);
     }
   };
 
   int64_t m = (int64_t)blockIdx.x * 32 + lane;
   for (int q = 0; q < kChipParts; ++q) {  // the first tile: every warp copies
-    if (q <= last) fill(m, role, q, 4);
+    if (q <= last) fill(m, role, q, nw, false);
     cp_commit();
   }
-  for (int k = threadIdx.x; k < 2 * N; k += kChipThreads) {
+  for (int k = threadIdx.x; k < 2 * N; k += T) {
     Rec* c = cs + (k < N ? k : NP - N + k);
 #pragma unroll
     for (int e = 0; e < Rec::W; ++e) c->v[e] = e <= P ? coef[k * (P + 1) + e] : 0.f;
@@ -89,15 +98,14 @@ sweep_chip_kernel(const float* __restrict__ coef, int N, int64_t M, int64_t ld, 
   struct Batch {
     float4 b[R / 4], c[CV];
   } A, B;
-  auto get = [&](Batch& t, const Rec* rec, int i0) {  // rows i0 .. i0+R-1
+  auto get = [&](Batch& t, const float4* p, const float4* c) {  // a batch's rows and coefficients
 #pragma unroll
-    for (int k = 0; k < R / 4; ++k) t.b[k] = col[((i0 >> 2) + k) * 32];
-    const float4* c = reinterpret_cast<const float4*>(rec + i0);
+    for (int k = 0; k < R / 4; ++k) t.b[k] = p[k * 32];
 #pragma unroll
     for (int k = 0; k < CV; ++k) t.c[k] = c[k];
   };
   // one batch of a sweep upwards (D = 1) or downwards (-1), in place in the tile
-  auto sweep = [&](const Batch& t, int i0, float& v1, float& v2, auto dir) {
+  auto sweep = [&](const Batch& t, float4* p, float& v1, float& v2, auto dir) {
     constexpr int D = decltype(dir)::value;
     Batch w = t;
     float* bv = reinterpret_cast<float*>(w.b);
@@ -111,42 +119,50 @@ sweep_chip_kernel(const float* __restrict__ coef, int N, int64_t M, int64_t ld, 
       v1 = v;
     }
 #pragma unroll
-    for (int k = 0; k < R / 4; ++k) col[((i0 >> 2) + k) * 32] = w.b[k];
+    for (int k = 0; k < R / 4; ++k) p[k * 32] = w.b[k];
   };
-  auto row = [&](const Rec* rec, int i, float& v1, float& v2, auto dir) {
-    const float v = F::step<P, (decltype(dir)::value > 0 ? F_ONE : B_ONE)>(rec[i].v, *at(i), v1, v2);
-    *at(i) = v;
+  auto row = [&](const Rec& c, float* p, float& v1, float& v2, auto dir) {
+    const float v = F::step<P, (decltype(dir)::value > 0 ? F_ONE : B_ONE)>(c.v, *p, v1, v2);
+    *p = v;
     v2 = v1;
     v1 = v;
   };
-  auto sweep_part = [&](int q, const Rec* rec, float& v1, float& v2, auto dir) {
+  // quarter q, whose rows lie `off` rows from their own places: whole batches, one read ahead,
+  // and the rows that are left over at its upper end
+  auto sweep_part = [&](int q, int off, const Rec* rec, float& v1, float& v2, auto dir) {
     constexpr int D = decltype(dir)::value;
-    const int lo = q * part, hi = end(q), nb = (hi - lo) / R, whole = lo + nb * R;
+    constexpr int ps = D * (R / 4) * 32, ks = D * CV;  // from a batch to the next one swept
+    const int lo = q * part, hi = end(q), whole = lo + (hi - lo) / R * R;
+    int nb = (hi - lo) / R;
     if constexpr (D < 0)
-      for (int i = hi - 1; i >= whole; --i) row(rec, i, v1, v2, dir);
-    auto first = [&](int k) { return lo + (D > 0 ? k : nb - 1 - k) * R; };  // of batch k
-    if (nb > 0) get(A, rec, first(0));
-    int k = 0;
-    for (; k + 2 < nb; k += 2) {
-      get(B, rec, first(k + 1));
-      sweep(A, first(k), v1, v2, dir);
-      get(A, rec, first(k + 2));
-      sweep(B, first(k + 1), v1, v2, dir);
+      for (int i = hi - 1; i >= whole; --i) row(rec[i], at(i + off), v1, v2, dir);
+    if (nb > 0) {
+      const int first = D > 0 ? lo : whole - R;
+      float4* p = col + ((first + off) >> 2) * 32;
+      const float4* c = reinterpret_cast<const float4*>(rec + first);
+      get(A, p, c);
+      for (; nb > 2; nb -= 2, p += 2 * ps, c += 2 * ks) {
+        get(B, p + ps, c + ks);
+        sweep(A, p, v1, v2, dir);
+        get(A, p + 2 * ps, c + 2 * ks);
+        sweep(B, p + ps, v1, v2, dir);
+      }
+      if (nb > 1) get(B, p + ps, c + ks);
+      sweep(A, p, v1, v2, dir);
+      if (nb > 1) sweep(B, p + ps, v1, v2, dir);
     }
-    if (k + 1 < nb) get(B, rec, first(k + 1));
-    if (k < nb) sweep(A, first(k), v1, v2, dir);
-    if (k + 1 < nb) sweep(B, first(k + 1), v1, v2, dir);
     if constexpr (D > 0)
-      for (int i = whole; i < hi; ++i) row(rec, i, v1, v2, dir);
+      for (int i = whole; i < hi; ++i) row(rec[i], at(i + off), v1, v2, dir);
   };
   using Up = std::integral_constant<int, 1>;
   using Down = std::integral_constant<int, -1>;
 
-  for (int64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x, m += (int64_t)gridDim.x * 32) {
-    // ---- forward, each quarter as it arrives
+  bool down = false;  // how this tile's quarters lie
+  for (int64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x, m += (int64_t)gridDim.x * 32, down = !down) {
+    // ---- forward, each quarter as it arrives (one group each, in order)
     float u1 = 0.f, u2 = 0.f;
     for (int q = 0; q <= last; ++q) {
-      if (tile != blockIdx.x || q == 3)
+      if (q == 3 || last != 3)
         cp_wait<0>();
       else if (q == 0)
         cp_wait<3>();
@@ -155,22 +171,24 @@ sweep_chip_kernel(const float* __restrict__ coef, int N, int64_t M, int64_t ld, 
       else
         cp_wait<1>();
       __syncthreads();
-      if (role == 0) sweep_part(q, cs, u1, u2, Up{});
+      if (role == 0) sweep_part(q, shift(q, down), cs, u1, u2, Up{});
     }
-    // ---- backward; a finished quarter is stored and refilled while the next one is swept
+    // ---- backward; a finished quarter is stored while the next one is swept, and its place
+    // takes quarter last - q of the next tile
     float x1 = 0.f, x2 = 0.f;
     const int64_t mn = m + (int64_t)gridDim.x * 32;
     for (int q = last; q >= 0; --q) {
-      if (role == 0) sweep_part(q, cs + NP, x1, x2, Down{});
+      if (role == 0) sweep_part(q, shift(q, down), cs + NP, x1, x2, Down{});
       __syncthreads();
       if (role != 0) {
         if (m < M) {
+          const int off = shift(q, down);
           TO* dst = x + m + (int64_t)(q * part + role - 1) * ld;
 #pragma unroll 4
-          for (int i = q * part + role - 1; i < end(q); i += 3, dst += 3 * ld)
-            st_stream(dst, Conv<F, TO>::out(*at(i)));
+          for (int i = q * part + role - 1; i < end(q); i += nw - 1, dst += (nw - 1) * ld)
+            st_stream(dst, Conv<F, TO>::out(*at(i + off)));
         }
-        if (tile + gridDim.x < ntiles) fill(mn, role - 1, q, 3);
+        if (tile + gridDim.x < ntiles) fill(mn, role - 1, last - q, nw - 1, !down);
         cp_commit();
       }
     }
@@ -178,21 +196,25 @@ sweep_chip_kernel(const float* __restrict__ coef, int N, int64_t M, int64_t ld, 
 }
 
 size_t chip_bytes(const sb_factor* f) {
-  const size_t rows = (f->N + 3) / 4 * 4;
-  return rows * (2 * (f->P == 1 ? sizeof(ChipRec<1>) : sizeof(ChipRec<2>)) + 32 * sizeof(float));
+  const size_t N = (size_t)f->N, part = (size_t)chip_part((int)f->N);
+  return (N + 3) / 4 * 4 * 2 * (f->P == 1 ? sizeof(ChipRec<1>) : sizeof(ChipRec<2>)) +
+         (N + part - 1) / part * part * 32 * sizeof(float);
 }
 
 template <int P, bool F_ONE, bool B_ONE, typename TO>
 int launch(const sb_factor* f, const float* coef, const float* rhs, TO* x, int64_t M, int64_t ld,
            cudaStream_t stream) {
   const size_t smem = chip_bytes(f);
-  auto k = sweep_chip_kernel<P, F_ONE, B_ONE, TO>;
+  // Seven copying warps where at most two tiles fit an SM: with an FP64 solution three take
+  // longer over a quarter than its sweep (N = 1000, M = 20001: 105 -> 92 us, FP32 86 -> 81).
+  const int threads = 3 * smem > (size_t)kMaxDynSmem ? 256 : 128;
+  auto k = threads == 256 ? sweep_chip_kernel<P, F_ONE, B_ONE, TO, 256> : sweep_chip_kernel<P, F_ONE, B_ONE, TO, 128>;
   int nb = 0;
-  SB_TRY(kernel_occupancy(reinterpret_cast<const void*>(k), f->device, kChipThreads, smem, &nb));
+  SB_TRY(kernel_occupancy(reinterpret_cast<const void*>(k), f->device, threads, smem, &nb));
   const int64_t ntiles = (M + 31) / 32;
   const int sms = std::max(1, sm_count(f->device));
   const int64_t grid = std::min<int64_t>(ntiles, (int64_t)nb * sms);
-  k<<<(unsigned)grid, kChipThreads, smem, stream>>>(coef, (int)f->N, M, ld, rhs, x, ntiles, sms);
+  k<<<(unsigned)grid, threads, smem, stream>>>(coef, (int)f->N, M, ld, rhs, x, ntiles, sms);
   return cuda_check(cudaGetLastError(), "on-chip sweep launch");
 }
 
@@ -207,9 +229,9 @@ bool chip_sweep_fits(const sb_factor* f, sb_dtype rt, sb_dtype xt, sb_arith arit
 // intermediate takes 8-byte places there.  With an FP32 solution those sweeps catch up once
 // they have enough warps to hide their latency and the intermediate still finds place in
 // L2: up to 16 warps an SM, or 10 where only one tile fits an SM (microseconds, sequential |
-// here: N = 256 M = 60001 52 | 41, M = 120001 77 | 82; N = 130 pentadiagonal M = 60001
-// 30 | 29, M = 120001 41 | 50; N = 1000 M = 20001 167 | 86, M = 60001 217 | 213,
-// pentadiagonal 225 | 242).
+// here with three copying warps: N = 256 M = 60001 52 | 41, M = 120001 77 | 82; N = 130
+// pentadiagonal M = 60001 30 | 29, M = 120001 41 | 50; N = 1000 M = 20001 167 | 86, M =
+// 60001 217 | 213, pentadiagonal 225 | 242).
 bool chip_sweep_applies(const sb_factor* f, sb_dtype rt, sb_dtype xt, int64_t M, sb_arith arith) {
   const int64_t warps = 2 * chip_bytes(f) <= (size_t)kMaxDynSmem ? 16 : 10;
   return chip_sweep_fits(f, rt, xt, arith) && M >= 1 &&
