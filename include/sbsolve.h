@@ -271,7 +271,8 @@ typedef struct {
  *     sweeps otherwise;
  *   FP32 right-hand sides: up to 128 rows the sequential sweeps with every system held in
  *     registers (the same bits), except that batches of at most two 32-system tiles an SM
- *     stay partitioned from 65 rows on; beyond 128 rows the partitioned solve.
+ *     stay partitioned from 65 rows on; beyond 128 rows the partitioned solve where its
+ *     alignment holds, else the sequential sweeps' bits.
  * These rules look at M and at the alignment of the call, and their forms eliminate in
  * different orders: the bits of a system's solution depend on the batch it is solved in (a
  * shard or a slice of a batch agrees with the whole to rounding).  SB_ALGO_SEQUENTIAL,
